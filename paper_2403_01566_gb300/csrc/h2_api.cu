@@ -660,13 +660,27 @@ static int write_dense(const double* d, const int* perm, const Tree& rows, const
   return H2_OK;
 }
 
-// Device copy of the orders of both trees (rows, then columns).
-static int upload_perm(const Tree& rows, const Tree& cols, int** d_perm) {
-  std::vector<int> p((size_t)rows.n + cols.n);
-  for (int64_t i = 0; i < rows.n; ++i) p[i] = (int)rows.perm[i];
-  for (int64_t i = 0; i < cols.n; ++i) p[rows.n + i] = (int)cols.perm[i];
-  CK(cudaMalloc(d_perm, p.size() * sizeof(int)));
-  CK(cudaMemcpy(*d_perm, p.data(), p.size() * sizeof(int), cudaMemcpyHostToDevice));
+// Device copy of the orders of both trees (rows, then columns), made on first
+// use.  Handles may be shared by host threads: `cached` is set under `mu`, and
+// only once the copy has arrived (the copy of pageable memory may return
+// earlier, and the library's streams do not wait for the legacy one).
+static int device_perm(const Tree& rows, const Tree& cols, std::mutex& mu, int*& cached, const int** out) {
+  std::lock_guard<std::mutex> lk(mu);
+  if (!cached) {
+    std::vector<int> p((size_t)rows.n + cols.n);
+    for (int64_t i = 0; i < rows.n; ++i) p[i] = (int)rows.perm[i];
+    for (int64_t i = 0; i < cols.n; ++i) p[rows.n + i] = (int)cols.perm[i];
+    int* d = nullptr;
+    CK(cudaMalloc(&d, p.size() * sizeof(int)));
+    cudaError_t e = cudaMemcpy(d, p.data(), p.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) {
+      cudaFree(d);
+      return cuda_fail(e, "orders of the clusters");
+    }
+    cached = d;
+  }
+  *out = cached;
   return H2_OK;
 }
 
@@ -708,6 +722,7 @@ struct h2_hmatrix {
   std::vector<int64_t> off_L, off_R;
   std::vector<int> w;
   int* d_int = nullptr;  // [rank of each admissible leaf][err]
+  mutable std::mutex mu;          // guards d_perm
   mutable int* d_perm = nullptr;  // orders of both trees, made on first use
   cudaEvent_t done = nullptr;
 };
@@ -1139,8 +1154,9 @@ int h2_hmatrix_to_dense(const h2_hmatrix* C, double* out, int on_device) {
   const double params[PARAM_COUNT] = {0.0, 0.0};
   rc = run_plan(rt, C->d_arena, nullptr, nullptr, nullptr, params, s, false);
   if (rc) return rc;
-  if (!C->d_perm && (rc = upload_perm(*C->rows, *C->cols, &C->d_perm))) return rc;
-  return write_dense(rt.d_ws, C->d_perm, *C->rows, *C->cols, out, on_device, s);
+  const int* perm;
+  if ((rc = device_perm(*C->rows, *C->cols, C->mu, C->d_perm, &perm))) return rc;
+  return write_dense(rt.d_ws, perm, *C->rows, *C->cols, out, on_device, s);
 }
 
 int h2_mul_profile(const h2_matrix* A, const h2_matrix* B, double eps, const h2_mul_opts* opts,
@@ -1213,7 +1229,8 @@ int h2_matvec_batch(const h2_matrix* Ac, const double* X, double* Y, int nrhs, i
   cudaStream_t s = stream ? (cudaStream_t)stream : g_stream;
   if (A->done) CK(cudaStreamWaitEvent(s, A->done, 0));
   const int64_t nr = A->rows->n, nc = A->cols->n;
-  if (!A->d_perm && (rc = upload_perm(*A->rows, *A->cols, &A->d_perm))) return rc;
+  const int* perm;
+  if ((rc = device_perm(*A->rows, *A->cols, A->mu, A->d_perm, &perm))) return rc;
   const MvKey key{matrix_sig(A), nrhs};
   std::shared_ptr<PlanRT> rt = mv_lookup(key);
   if (!rt) {
@@ -1237,7 +1254,7 @@ int h2_matvec_batch(const h2_matrix* Ac, const double* X, double* Y, int nrhs, i
     Yd = stage + (size_t)nc * nrhs;
   }
   const int64_t nx = nc * nrhs, ny = nr * nrhs;
-  k_perm_gather<<<(unsigned)std::min<int64_t>((nx + 255) / 256, 65535 * 8), 256, 0, s>>>(Xd, A->d_perm + nr, nc,
+  k_perm_gather<<<(unsigned)std::min<int64_t>((nx + 255) / 256, 65535 * 8), 256, 0, s>>>(Xd, perm + nr, nc,
                                                                                          nrhs, Xc);
   if (P.ext_slots)  // the ranks of a product
     CK(cudaMemcpyAsync(rt->d_slot, A->d_int, sizeof(int) * P.slot_init.size(), cudaMemcpyDeviceToDevice, s));
@@ -1247,7 +1264,7 @@ int h2_matvec_batch(const h2_matrix* Ac, const double* X, double* Y, int nrhs, i
     if (stage) cudaFreeAsync(stage, s);
     return rc;
   }
-  k_perm_scatter<<<(unsigned)std::min<int64_t>((ny + 255) / 256, 65535 * 8), 256, 0, s>>>(Yc, A->d_perm, nr, nrhs,
+  k_perm_scatter<<<(unsigned)std::min<int64_t>((ny + 255) / 256, 65535 * 8), 256, 0, s>>>(Yc, perm, nr, nrhs,
                                                                                           Yd);
   CK(cudaEventRecord(rt->last, s));
   if (!on_device) {
@@ -1276,8 +1293,9 @@ int h2_to_dense(const h2_matrix* Ac, double* out, int on_device) {
   const double params[PARAM_COUNT] = {0.0, 0.0};
   rc = run_plan(rt, A->d_arena, nullptr, nullptr, nullptr, params, s, false);
   if (rc) return rc;
-  if (!A->d_perm && (rc = upload_perm(*A->rows, *A->cols, &A->d_perm))) return rc;
-  return write_dense(rt.d_ws, A->d_perm, *A->rows, *A->cols, out, on_device, s);
+  const int* perm;
+  if ((rc = device_perm(*A->rows, *A->cols, A->mu, A->d_perm, &perm))) return rc;
+  return write_dense(rt.d_ws, perm, *A->rows, *A->cols, out, on_device, s);
 }
 
 }  // extern "C"
