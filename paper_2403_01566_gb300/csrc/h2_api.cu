@@ -626,8 +626,9 @@ __global__ void __launch_bounds__(256) k_perm_dense(const double* __restrict__ d
 // order, then the columns' (device).  Runs on stream s, after the work of the
 // legacy default stream on `out`, and waits for it.  (On the host, with two
 // copies of the matrix, the reordering took 26 of the 30 ms of an expanded
-// H-matrix product of n = 2025.)  Host output without room for a second device
-// copy of the matrix is reordered on the host.
+// H-matrix product of n = 2025.)  The temporary of a host output is not taken
+// from the stream's pool, which would keep it after the call; without room for
+// it the matrix is reordered on the host.
 static int write_dense(const double* d, const int* perm, const Tree& rows, const Tree& cols, double* out,
                        int on_device, cudaStream_t s) {
   const int64_t nr = rows.n, nc = cols.n;
@@ -639,7 +640,7 @@ static int write_dense(const double* d, const int* perm, const Tree& rows, const
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev, 0);
     cudaEventDestroy(ev);
     if (e != cudaSuccess) return cuda_fail(e, "dense expansion");
-  } else if (cudaMallocAsync(&o, (size_t)nr * nc * sizeof(double), s) != cudaSuccess) {
+  } else if (cudaMalloc(&o, (size_t)nr * nc * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     std::vector<double> h((size_t)nr * nc);
     CK(cudaStreamSynchronize(s));
@@ -653,9 +654,9 @@ static int write_dense(const double* d, const int* perm, const Tree& rows, const
   cudaError_t e = cudaGetLastError();
   if (!on_device) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, o, (size_t)nr * nc * sizeof(double), cudaMemcpyDeviceToHost, s);
-    cudaFreeAsync(o, s);
   }
   const cudaError_t e2 = cudaStreamSynchronize(s);
+  if (!on_device) cudaFree(o);
   if (e != cudaSuccess || e2 != cudaSuccess) return cuda_fail(e != cudaSuccess ? e : e2, "dense expansion");
   return H2_OK;
 }
