@@ -91,6 +91,7 @@ struct PlanRT {
   double* d_ws = nullptr;
   cudaGraphExec_t graph = nullptr;
   cudaEvent_t last = nullptr;  // completion of the last replay (workspace reuse)
+  std::mutex mu;               // held while a replay is enqueued (header, workspace and `last` are shared)
   int nrank = 0;
   // pinned ring of control headers (asynchronous upload without a host wait)
   static constexpr int RING = 64;
@@ -980,8 +981,10 @@ static int enqueue_product(const MulArgs& m, PlanRT& rt, cudaStream_t s, h2_kern
   if ((rc = new_product_matrix(m, *rt.plan, s, &C))) return rc;
   double params[PARAM_COUNT];
   product_params(m, params);
+  std::unique_lock<std::mutex> lk(rt.mu);
   rc = prof ? run_plan_profiled(rt, A->d_arena, B->d_arena, C->d_arena, C->d_int, params, s, prof)
             : run_plan(rt, A->d_arena, B->d_arena, C->d_arena, C->d_int, params, s, true);
+  lk.unlock();
   if (rc) {
     h2_free(C);
     return rc;
@@ -1089,7 +1092,10 @@ static int hmul_impl(const h2_matrix* Ac, const h2_matrix* Bc, double eps, const
   cudaMemsetAsync(C->d_arena, 0, C->arena_len * sizeof(double), s);
   cudaMemsetAsync(C->d_int, 0, nint * sizeof(int), s);
   const double params[PARAM_COUNT] = {0.0, eps / 3.0, svd_noise_floor(eps, 0)};
-  rc = run_plan(*rt, A->d_arena, B->d_arena, C->d_arena, C->d_int, params, s, true);
+  {
+    std::lock_guard<std::mutex> lk(rt->mu);
+    rc = run_plan(*rt, A->d_arena, B->d_arena, C->d_arena, C->d_int, params, s, true);
+  }
   if (rc) {
     h2_hmatrix_free(C);
     return rc;
@@ -1241,7 +1247,9 @@ int h2_matvec_batch(const h2_matrix* Ac, const double* X, double* Y, int nrhs, i
     mv_insert(key, rt);
   }
   const Plan& P = *rt->plan;
-  // the plan's workspace is shared by its replays: order this call after the last
+  // the plan's workspace is shared by its replays: order this call after the
+  // last, and keep other threads' calls out until this one is enqueued
+  std::unique_lock<std::mutex> lk(rt->mu);
   CK(cudaStreamWaitEvent(s, rt->last, 0));
   double* Xc = rt->d_ws + P.mv_ox;
   double* Yc = rt->d_ws + P.mv_oy;
@@ -1268,6 +1276,7 @@ int h2_matvec_batch(const h2_matrix* Ac, const double* X, double* Y, int nrhs, i
   k_perm_scatter<<<(unsigned)std::min<int64_t>((ny + 255) / 256, 65535 * 8), 256, 0, s>>>(Yc, perm, nr, nrhs,
                                                                                           Yd);
   CK(cudaEventRecord(rt->last, s));
+  lk.unlock();
   if (!on_device) {
     CK(cudaMemcpyAsync(Y, Yd, (size_t)nr * nrhs * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaFreeAsync(stage, s));
