@@ -208,7 +208,7 @@ static int run_plan(PlanRT& rt, double* bx, double* by, double* bc, int* out_int
       cudaMemcpyAsync(rt.d_slot, rt.d_slot_init, sizeof(int) * P.slot_init.size(), cudaMemcpyDeviceToDevice, cs);
     cudaMemsetAsync(rt.d_err, 0, sizeof(int), cs);
     for (const Stage& st : P.stages) launch_stage(st, rt.d_ctx, rt.dj, cs);
-    if (rt.nrank) launch_finalize(rt.d_ctx, rt.nrank, cs);
+    if (P.reports) launch_finalize(rt.d_ctx, rt.nrank, cs);
     cudaError_t e = cudaStreamEndCapture(cs, &g);
     cudaStreamDestroy(cs);
     if (e != cudaSuccess) return cuda_fail(e, "capture");
@@ -223,7 +223,7 @@ static int run_plan(PlanRT& rt, double* bx, double* by, double* bc, int* out_int
       CK(cudaMemcpyAsync(rt.d_slot, rt.d_slot_init, sizeof(int) * P.slot_init.size(), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemsetAsync(rt.d_err, 0, sizeof(int), s));
     for (const Stage& st : P.stages) launch_stage(st, rt.d_ctx, rt.dj, s);
-    launch_finalize(rt.d_ctx, rt.nrank, s);
+    if (P.reports) launch_finalize(rt.d_ctx, rt.nrank, s);
   }
   CK(cudaGetLastError());
   CK(cudaEventRecord(rt.last, s));

@@ -58,6 +58,8 @@ struct Plan {
   int64_t fac_len = 0;           // doubles of the terminal-factor arena (placed after the workspace)
   int64_t mv_ox = 0, mv_oy = 0;  // matrix-vector plans: X and Y in the workspace
   bool ext_slots = false;        // the caller sets the slots before a replay
+  bool reports = false;          // a product: its replays end by writing its ranks (there may be none) and its
+                                 // error flag to the caller's integer array
   // H-matrix output (MulOptions::hmatrix): per admissible leaf of the target
   // block tree (adm_list order) the factors L (|t| x w) and R (|r| x w) in the
   // product arena, zero-padded to the width cap w; their ranks go to the
