@@ -38,6 +38,19 @@ constexpr int SVD_SMALL_DOUBLES = 5120;
 H2_HOST_DEVICE constexpr int svd_colarr_doubles(int cmax) {
   return 4 * cmax + 2 * (cmax / 2 + 1) + (cmax + cmax / 2 + 2) / 2 + 1;
 }
+// Whether a CTA of `threads` takes a job of `cols` columns: every column has a
+// thread (its norm), and the warps that hold the pairs, one per 64 columns,
+// leave a warp for the rows.
+H2_HOST_DEVICE constexpr bool svd_cta_takes(int cols, int threads) {
+  return cols <= threads && (cols + 63) / 64 < threads / 32;
+}
+// Shared memory of a job in doubles (0: empty).  One that the CTAs of small
+// jobs (128 threads) do not take counts as larger than those.
+H2_HOST_DEVICE constexpr int64_t svd_need_doubles(int rows, int cols) {
+  if (rows <= 0 || cols <= 0) return 0;
+  const int64_t need = svd_colarr_doubles(cols) + (int64_t)(rows + 1) * cols;
+  return need <= SVD_SMALL_DOUBLES && !svd_cta_takes(cols, 128) ? SVD_SMALL_DOUBLES + 1 : need;
+}
 constexpr int GEMM_MAXTILE = 64; // largest GEMM output tile (rows and columns)
 
 // Device copies of the job arrays of a stage list.
