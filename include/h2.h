@@ -72,10 +72,13 @@ typedef struct {
  *              (binary trees); 0 selects 1/4
  *   max_rank   cap on the adaptive ranks (storage padding of C), <= 64; 0 selects
  *              min(64, max(32, 2k))
- *   precision  0 = FP64 throughout (the GEMM stages of 64 x 64 tiles as exact
+ *   precision  0 = FP64 throughout (the GEMM stages of 64 x 64 tiles as
  *                  integer slices of the FP64 operands on the tensor cores, 62
- *                  bits of each operand, FP64 sums: the error of an FP64
- *                  product or less);
+ *                  bits of each operand relative to its row's or column's
+ *                  largest entry, FP64 sums.  Every entry of a product of
+ *                  matrix data is within FP64's bound, relative to |A| |B|;
+ *                  block factors, which pass through a QR or an SVD, are
+ *                  relative to the largest entries of their rows and columns);
  *              1 = FP32 contractions: the accumulation phases (basis products,
  *                  coupling and nearfield products, splits and pushes; Sections
  *                  3-4) and the coupling projection (Section 5.2) compute FP32
@@ -87,8 +90,8 @@ typedef struct {
  *              2 = compensated FP32 contractions: operands split into FP32
  *                  hi + lo parts, error-free products and compensated sums
  *                  (about 1e-13 relative); the GEMM stages of 64 x 64 tiles as
- *                  in form 0, which is faster there and no less accurate; QR,
- *                  SVD, rank decisions and norms stay FP64.
+ *                  in form 0, which is faster there; QR, SVD, rank decisions
+ *                  and norms stay FP64.
  *              3 = every GEMM stage on the tensor cores (FP16 integer slices,
  *                  FP32 accumulation) with 5 slices of 8 bits per operand
  *                  (row and column scaled per k chunk of 32; exact FP32 sums
