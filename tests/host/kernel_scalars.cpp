@@ -50,4 +50,18 @@ void pair_tan(double na, double nb, float g, float* t) {
   t[1] = h2::jacobi_tan(g, d, h2::jacobi_threshold(nb, na));
 }
 float threshold(double na, double nb) { return h2::jacobi_threshold(na, nb); }
+
+void reciprocals(const double* v, int n, double* rsq, double* rec) {
+  for (int i = 0; i < n; ++i) {
+    rsq[i] = h2::rsqrt_pos(v[i]);
+    rec[i] = h2::recip_pos(v[i]);
+  }
+}
+// q = 1 + t^2 and 1 / sqrt(q) of a rotation
+void cosines(const float* t, int n, double* q, double* c) {
+  for (int i = 0; i < n; ++i) {
+    q[i] = fma((double)t[i], (double)t[i], 1.0);
+    c[i] = h2::jacobi_cos(q[i], t[i]);
+  }
+}
 }
