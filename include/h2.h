@@ -272,7 +272,7 @@ void h2_server_destroy(h2_server* s);
  *   h2_batch_info     launches per run (scans counted per product), persistent
  *                     chains among them, kernel launches of the last enqueue
  *   h2_batch_autotune times every GEMM launch of the batch with each kernel
- *                     variant (outputs per thread, tiles per warp) and, for
+ *                     variant (outputs per thread; the tensor-core form has one) and, for
  *                     chains, CTAs per SM, pins the fastest per shape class in
  *                     a process-wide table used by batches created afterwards,
  *                     and re-captures this batch; the choices never change a

@@ -1619,7 +1619,7 @@ namespace h2 {
 namespace {
 
 // Pinned launch choices of the autotuner per GEMM shape class: kernel
-// variant (outputs per thread or tiles per warp) and, for persistent chains,
+// variant (outputs per thread; the tensor-core form has one) and, for persistent chains,
 // CTAs per SM.  Neither changes the arithmetic of a job.
 struct TuneKey {
   int mode, slices, mmax, nb, chain;
